@@ -164,8 +164,9 @@ int cutqc_attribute_noalloc(const cutqc_subcircuit* s, const void* variants_dev,
  *
  * out_dev: float32 output in out_order (KRON or ORIGINAL).  Rows
  * [row_begin, row_end) of the final contraction are written, where a row is
- * one value of the high output bits (the operand that the final step puts in
- * the rows); row_end = -1 means all rows.  With a partial range the output
+ * one value of the output bits of the operand that holds the highest output
+ * bit in out_order; row_end = -1, or that operand's row count (cutqc_fd_shape
+ * gives it for KRON), means all rows.  With a partial range the output
  * must be in KRON order and out_dev receives indices
  * [row_begin * cols, row_end * cols) (cols from cutqc_fd_shape) starting at
  * out_dev[0].  This is the offset/stride split used to shard one

@@ -129,6 +129,8 @@ struct ContractionPlan {
   int K = 0;                          // number of distinct cut edges
   int n = 0;                          // output bits
   size_t ws_bytes = 0;                // per batch item
+  // rows and columns of a row range: the last step with the highest output
+  // bit in its rows (low_to_cols may give the step the other way round)
   int64_t final_rows = 1, final_cols = 1;
 };
 
@@ -154,7 +156,8 @@ int plan_contraction_batched(const std::vector<TensorDesc>& inputs, int precisio
 // inputs[i] + b * in_bstride[i]; output of item b at out + b * out_bstride;
 // sum + b (if sum).  Workspace: plan.ws_bytes * batch.  in_ready (nullable):
 // one event per input (null entries allowed) that the steps reading that
-// input wait for on their stream.
+// input wait for on their stream.  row_begin, row_end: rows of the last
+// step's row operand (row_end < 0: all of them).
 int run_plan(const ContractionPlan& plan, const float* const* inputs, const int64_t* in_bstride, int batch,
              float* out, int64_t out_bstride, double* sum, float alpha, int precision, int64_t row_begin,
              int64_t row_end, uint8_t* ws, cudaStream_t st, const cudaEvent_t* in_ready = nullptr);

@@ -200,6 +200,10 @@ int plan_contraction_batched(const std::vector<TensorDesc>& inputs, int precisio
       int ma = A.o ? *std::max_element(A.pos.begin(), A.pos.end()) : -1;
       int mb = B.o ? *std::max_element(B.pos.begin(), B.pos.end()) : -1;
       if (mb > ma) std::swap(best_a, best_b);
+      // the rows of a row range (cutqc_fd_shape), whichever operand of the
+      // step they become below
+      plan->final_rows = (int64_t)1 << plan->tensors[best_a].o;
+      plan->final_cols = (int64_t)1 << plan->tensors[best_b].o;
       // low_to_cols: the operand holding the lowest output bit goes to the
       // columns instead (runs of consecutive columns are then runs of
       // consecutive floats), whichever holds the highest
@@ -254,8 +258,6 @@ int plan_contraction_batched(const std::vector<TensorDesc>& inputs, int precisio
       for (int b = 0; b < B.o; ++b) mn |= (uint64_t)1 << B.pos[b];
       st.mask_m = mm;
       st.mask_n = mn;
-      plan->final_rows = st.M;
-      plan->final_cols = st.N;
       R.pos = B.pos;
       R.pos.insert(R.pos.end(), A.pos.begin(), A.pos.end());
     } else {
@@ -376,8 +378,10 @@ int run_plan(const ContractionPlan& plan, const float* const* inputs, const int6
     CUTQC_LAUNCH_CHECK("single_copy");
     return CUTQC_OK;
   }
-  if (row_end < 0) row_end = plan.final_rows;
-  const bool partial = row_begin != 0 || row_end != plan.final_rows;
+  // row_end < 0: every row of the last step's row operand
+  const int64_t all_rows = plan.stages.back().M;
+  if (row_end < 0) row_end = all_rows;
+  const bool partial = row_begin != 0 || row_end != all_rows;
   auto src_of = [&](int t, int64_t* bstride) -> const float* {
     if (t < (int)n_in) {
       *bstride = in_bstride[t];
@@ -797,7 +801,7 @@ extern "C" int cutqc_reconstruct_fd(int n_sub, const cutqc_subcircuit* s, const 
   if (rc) return rc;
   ContractionPlan plan;
   // uncut qubit order: either operand of the last step may hold the low
-  // output bits, and a row range is never asked for
+  // output bits, and only the whole row range is served
   if ((rc = plan_contraction(in, precision, &plan, out_order == CUTQC_ORDER_ORIGINAL))) return rc;
   if (!attributed || !out) return set_error(CUTQC_EINVAL, "null pointer");
   for (int i = 0; i < n_sub; ++i)
@@ -819,5 +823,5 @@ extern "C" int cutqc_reconstruct_fd(int n_sub, const cutqc_subcircuit* s, const 
   }
   std::vector<int64_t> bstride(n_sub, 0);
   return run_plan(plan, attributed, bstride.data(), 1, out, 0, sum, std::ldexp(1.0f, -plan.K), precision, row_begin,
-                  row_end, (uint8_t*)ws_dev, (cudaStream_t)stream, ready.empty() ? nullptr : ready.data());
+                  partial ? row_end : -1, (uint8_t*)ws_dev, (cudaStream_t)stream, ready.empty() ? nullptr : ready.data());
 }

@@ -2,6 +2,7 @@
 that include/cutqc.h declares.  No compute calls here."""
 import ctypes
 import subprocess
+import types
 
 import pytest
 
@@ -260,3 +261,28 @@ def test_fd_input_events_host_checks(built):
     # cleared by that call: the next one fails on the output order instead
     assert call() == cutqc.EINVAL
     assert "out_order" in cutqc.cutqc_last_error()
+
+
+def test_uncut_order_rows_are_those_of_the_highest_bit(built):
+    """In uncut qubit order the row count of a full range is that of the
+    operand holding the highest output bit, also where the last step takes
+    that operand as its columns (it holds output bit 0 too).  Every call
+    fails on the host: one row fewer is a partial range, which needs
+    Kronecker order; one more is outside the range; nothing reaches a launch."""
+    import torch
+    cq = built
+    qa = [0, 1, 2] + list(range(13, 22))
+    a = _sub(16, out_local=range(12, 16), out_edge=range(4), out_qubit=qa)
+    b = _sub(10, in_local=range(4), in_edge=range(4), out_qubit=range(3, 13))
+    rows, cols = cq.cutqc_fd_shape([a, b])
+    assert (rows, cols) == (4096, 1024)
+    att = [torch.zeros(1), torch.zeros(1)]          # host stand-ins: not dereferenced here
+    out = torch.zeros(1)
+    null = types.SimpleNamespace(cuda_stream=0)
+    for prec in (cq.PREC_FP32_SIMT, cq.PREC_FP16X3_TC, cq.PREC_FP16X3_TC_PRUNE):
+        ws = torch.empty(cq.cutqc_reconstruct_fd_workspace_size([a, b], prec), dtype=torch.uint8)
+        for row_end, text in ((rows - 1, "needs CUTQC_ORDER_KRON"), (cols, "needs CUTQC_ORDER_KRON"),
+                              (rows + 1, "outside [0, 4096)")):
+            with pytest.raises(cq.CutqcError) as e:
+                cq.cutqc_reconstruct_fd([a, b], att, cq.ORDER_ORIGINAL, prec, 0, row_end, out=out, ws=ws, stream=null)
+            assert e.value.code == cq.EINVAL and text in str(e.value)

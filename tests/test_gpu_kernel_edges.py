@@ -424,3 +424,19 @@ def test_dependent_launches_in_graphs_and_on_streams(cq, oa, ob, k):
     for i, (att, out, ws) in enumerate(sets):
         assert torch.equal(out, eager[i])
     assert cq.cutqc_device_status() == 0
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+def test_whole_row_range_in_uncut_order(cq, precision):
+    """The whole row range given by its end, for the operand of the highest
+    output bit in the rows and (it holds output bit 0 too) in the columns of
+    the last step: the result of row_end = -1."""
+    import torch
+    dev, _ = _operands(torch, 12, 10, 4, 3)
+    for qa in (list(range(10, 22)), [0, 1, 2] + list(range(13, 22))):
+        subs, _, _ = _pair(12, 10, 4, qa)
+        rows, _ = cq.cutqc_fd_shape(subs)
+        whole, _ = cq.cutqc_reconstruct_fd(subs, dev, cq.ORDER_ORIGINAL, precision)
+        out = torch.full_like(whole, 7.0)
+        cq.cutqc_reconstruct_fd(subs, dev, cq.ORDER_ORIGINAL, precision, 0, rows, out=out)
+        assert torch.equal(out, whole)
