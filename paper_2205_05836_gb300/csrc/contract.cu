@@ -987,13 +987,15 @@ sgemm64_kernel(const __grid_constant__ Sg128Args g, int64_t a_bstride, int64_t b
                g.sum ? g.sum + blockIdx.z : nullptr, g.streaming, blockIdx.y, blockIdx.x, sm);
 }
 
+bool sgemm_rows_supported(int64_t rows) { return (rows + SG_BM - 1) / SG_BM <= 65535; }
+
 int launch_sgemm(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t M, int64_t N,
                  int64_t K, float alpha, uint64_t mask_m, uint64_t mask_n, float* out, double* sum,
                  int streaming, cudaStream_t st, int batch, int64_t a_bstride, int64_t b_bstride,
                  int64_t out_bstride) {
   if (M <= 0 || N <= 0) return CUTQC_OK;
   int64_t gm = (M + SG_BM - 1) / SG_BM, gn = (N + SG_BN - 1) / SG_BN;
-  if (gm > 65535) return set_error(CUTQC_EUNSUPPORTED, "too many row tiles (%lld)", (long long)gm);
+  if (!sgemm_rows_supported(M)) return set_error(CUTQC_EUNSUPPORTED, "too many row tiles (%lld)", (long long)gm);
   if (gn > 0x7fffffff) return set_error(CUTQC_EUNSUPPORTED, "too many column tiles");
   if (batch < 1 || batch > 65535) return set_error(CUTQC_EUNSUPPORTED, "batch %d out of range", batch);
   Sg128Args g{};

@@ -73,6 +73,8 @@ int launch_prune_select(const OperandView& va, const int* a_bits, int a_nbits, i
 // float32 CUDA-core GEMM with bit-deposit epilogue.
 // batch > 1: item b uses A + b*a_bstride, B + b*b_bstride, out + b*out_bstride,
 // sum + b.
+// sgemm_rows_supported: its row tiles fit the grid's second dimension.
+bool sgemm_rows_supported(int64_t rows);
 int launch_sgemm(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t M, int64_t N,
                  int64_t K, float alpha, uint64_t mask_m, uint64_t mask_n, float* out, double* sum,
                  int streaming, cudaStream_t st, int batch = 1, int64_t a_bstride = 0, int64_t b_bstride = 0,

@@ -206,8 +206,12 @@ int plan_contraction_batched(const std::vector<TensorDesc>& inputs, int precisio
       plan->final_cols = (int64_t)1 << plan->tensors[best_b].o;
       // low_to_cols: the operand holding the lowest output bit goes to the
       // columns instead (runs of consecutive columns are then runs of
-      // consecutive floats), whichever holds the highest
-      if (low_to_cols) {
+      // consecutive floats), whichever holds the highest.  The FP32 GEMM
+      // takes fewer rows than columns (its row tiles are a grid's second
+      // dimension): operands past that keep their places
+      const bool movable = precision != CUTQC_PREC_FP32_SIMT ||
+                           (sgemm_rows_supported(plan->final_rows) && sgemm_rows_supported(plan->final_cols));
+      if (low_to_cols && movable) {
         const TensorDesc& R = plan->tensors[best_a];
         if (R.o && *std::min_element(R.pos.begin(), R.pos.end()) == 0) std::swap(best_a, best_b);
       }

@@ -440,3 +440,19 @@ def test_whole_row_range_in_uncut_order(cq, precision):
         out = torch.full_like(whole, 7.0)
         cq.cutqc_reconstruct_fd(subs, dev, cq.ORDER_ORIGINAL, precision, 0, rows, out=out)
         assert torch.equal(out, whole)
+
+
+def test_fp32_columns_past_the_row_limit_in_uncut_order(cq):
+    """A row operand of few outputs that holds the lowest and the highest
+    output bit against 2^24 columns (more than the FP32 GEMM takes as rows).
+    Bound: the float32 chain, (4 + 2) 2^-24 of the absolute terms."""
+    import torch
+    dev, _ = _operands(torch, 3, 24, 1, 9)
+    subs, _, _ = _pair(3, 24, 1, [0, 1, 26])
+    out, _ = cq.cutqc_reconstruct_fd(subs, dev, cq.ORDER_ORIGINAL, cq.PREC_FP32_SIMT)
+    A, B = (x.double() for x in dev)
+    got = out.view(2, 1 << 24, 4)
+    for top in range(2):
+        a = A[4 * top:4 * top + 4]
+        err = (got[top].double() - B @ a.T / 2).abs()
+        assert bool((err <= 6 * 2.0 ** -24 * (B.abs() @ a.abs().T) / 2).all())
