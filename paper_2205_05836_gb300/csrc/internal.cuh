@@ -157,6 +157,38 @@ __device__ __forceinline__ float2 unpack2(unsigned long long v) {
   return f;
 }
 
+// A float32 sum that carries its rounding errors beside it (Knuth's two-sum:
+// each step's error is exact), for totals that go on in float64.  A float64
+// add per group of outputs is exact too, but GB300's FP64 pipe takes a few
+// lanes per clock.  Terms up to the float32 range over their number.
+struct Sum2 {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
+    s = t;
+  }
+  // (after an infinity or a NaN the errors mean nothing)
+  __device__ __forceinline__ double value() const { return isfinite(s) ? (double)s + (double)e : (double)s; }
+};
+// Two of them in the halves of packed registers.
+struct Sum2x2 {
+  unsigned long long s = 0ull, e = 0ull;
+  static __device__ __forceinline__ unsigned long long sub(unsigned long long a, unsigned long long b) {
+    return fadd2(a, b ^ 0x8000000080000000ull);
+  }
+  __device__ __forceinline__ void add(unsigned long long v) {
+    const unsigned long long t = fadd2(s, v), b = sub(t, s);
+    e = fadd2(e, fadd2(sub(s, sub(t, b)), sub(v, b)));
+    s = t;
+  }
+  __device__ __forceinline__ double value() const {
+    const float2 a = unpack2(s), b = unpack2(e);
+    return (isfinite(a.x) ? (double)a.x + (double)b.x : (double)a.x) +
+           (isfinite(a.y) ? (double)a.y + (double)b.y : (double)a.y);
+  }
+};
+
 // Software bit deposit: scatter the low bits of v to the set bits of mask.
 __host__ __device__ __forceinline__ uint64_t pdep64(uint64_t v, uint64_t mask) {
   uint64_t r = 0;

@@ -456,3 +456,27 @@ def test_fp32_columns_past_the_row_limit_in_uncut_order(cq):
         a = A[4 * top:4 * top + 4]
         err = (got[top].double() - B @ a.T / 2).abs()
         assert bool((err <= 6 * 2.0 ** -24 * (B.abs() @ a.abs().T) / 2).all())
+
+
+# Equal outputs: every add of a float32 chain then rounds the same way.
+_EQUAL = (1.1, 1.3, 1.7, 0.7)
+
+
+@pytest.mark.parametrize("oa,ob,k", [(14, 8, 0), (14, 8, 2), (12, 10, 1), (11, 11, 0), (10, 12, 1), (9, 14, 0), (8, 14, 1),
+                                     (7, 15, 2)])
+def test_outer_product_totals_of_equal_outputs(cq, oa, ob, k):
+    """The float64 total of outer-product steps at every width of its tiles
+    (one, two and four column groups per thread, one to sixteen rows at a
+    time): at most 8 outputs are added in float32 (three roundings), the rest
+    without rounding but for the float64 adds."""
+    import torch
+    subs, _, _ = _pair(oa, ob, k)
+    for c in _EQUAL:
+        A = torch.zeros((1 << oa, 4 ** k), device="cuda")
+        B = torch.zeros((1 << ob, 4 ** k), device="cuda")
+        A[:, 0], B[:, 0] = c, 2.0 ** k
+        total = torch.zeros(1, dtype=torch.float64, device="cuda")
+        out, _ = cq.cutqc_reconstruct_fd(subs, [A, B], cq.ORDER_KRON, cq.PREC_FP32_SIMT, sum_out=total)
+        ref = out.double().sum().item()
+        assert abs(ref - out.numel() * float(np.float32(c))) <= 1e-9 * ref
+        assert abs(total.item() - ref) <= 3 * 2.0 ** -24 * ref, c
