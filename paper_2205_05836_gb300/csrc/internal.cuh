@@ -168,6 +168,10 @@ struct Sum2 {
     e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
     s = t;
   }
+  __device__ __forceinline__ void add(const Sum2& o) {
+    add(o.s);
+    e = __fadd_rn(e, o.e);
+  }
   // (after an infinity or a NaN the errors mean nothing)
   __device__ __forceinline__ double value() const { return isfinite(s) ? (double)s + (double)e : (double)s; }
 };

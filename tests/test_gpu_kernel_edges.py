@@ -480,3 +480,54 @@ def test_outer_product_totals_of_equal_outputs(cq, oa, ob, k):
         ref = out.double().sum().item()
         assert abs(ref - out.numel() * float(np.float32(c))) <= 1e-9 * ref
         assert abs(total.item() - ref) <= 3 * 2.0 ** -24 * ref, c
+
+
+def _uneven(torch, oa, ob, k, big, small):
+    """Operands whose product's rows are all 1 (where big(row)) or all
+    `small`."""
+    A = torch.zeros((1 << oa, 4 ** k), device="cuda")
+    B = torch.zeros((1 << ob, 4 ** k), device="cuda")
+    m = torch.arange(1 << oa, device="cuda")
+    A[:, 0] = torch.where(big(m), 1.0, small)
+    B[:, 0] = 2.0 ** k
+    return A, B
+
+
+@pytest.mark.parametrize("oa,ob,k,original,rounds", [(12, 11, 3, False, 3), (12, 11, 3, True, 3), (11, 12, 4, False, 3),
+                                                     (13, 6, 4, False, 2), (6, 13, 4, True, 2)])
+def test_fp32_gemm_totals_of_uneven_rows(cq, oa, ob, k, original, rounds):
+    """The float64 total of FP32 steps in 128 x 128 tiles (16-byte and single
+    stores) and 64 x 64 tiles, where the first of a thread's rows is 1 and the
+    others are just below half the last place of four (or sixteen) ones: at
+    most 8 and 4 outputs, of one row, are added in float32 (three and two
+    roundings), the rest without rounding but for the float64 adds."""
+    import torch
+    n = oa + ob
+    subs, _, _ = _pair(oa, ob, k, [2 * i + 1 for i in range(oa - 1)] + [n - 1] if original else None)
+    A, B = _uneven(torch, oa, ob, k, lambda m: (m % 4 == 0) & (m // 64 % 2 == 0), 2.0 ** -24 * (1 - 2.0 ** -6))
+    total = torch.zeros(1, dtype=torch.float64, device="cuda")
+    out, _ = cq.cutqc_reconstruct_fd(subs, [A, B], cq.ORDER_ORIGINAL if original else cq.ORDER_KRON, cq.PREC_FP32_SIMT,
+                                     sum_out=total)
+    ref = (A[:, 0].double().sum() * 2.0 ** ob).item()
+    assert abs(out.double().sum().item() - ref) <= 1e-12 * ref
+    assert abs(total.item() - ref) <= rounds * 2.0 ** -24 * ref
+
+
+@pytest.mark.parametrize("narrow", [-1, 16])
+def test_dd_bin_totals_of_uneven_rows(cq, narrow):
+    """The same for the bin totals of the level launches and of the persistent
+    launch's 64 x 64 and 256 x 16 tiles: four bins of one row are added in
+    float32 (two roundings), the rest without rounding but for the float64
+    adds."""
+    import torch
+    subs, _, _ = _pair(8, 4, 1)
+    A, B = _uneven(torch, 8, 4, 1, lambda m: m % 4 == 0, 2.0 ** -24 * (1 - 2.0 ** -6))
+    run = cq.dd_batch_run(subs, [A, B], 12, 12, 1, 1, max_jobs=4)
+    cq.cutqc_dd_batch_create([run], options={"narrow_max_n": narrow}).launch()
+    jobs, n_jobs, bins = cq.cutqc_dd_run_async(subs, [A, B], 12, 12, 1, 1)
+    torch.cuda.synchronize()
+    ref = (A[:, 0].double().sum() * 2.0 ** 4).item()
+    for J, b in ((cq.dd_jobs_from_device(run["jobs"], run["n_jobs"])[0], run["bins"]),
+                 (cq.dd_jobs_from_device(jobs, n_jobs)[0], bins)):
+        assert abs(b[:1 << 12].double().sum().item() - ref) <= 1e-12 * ref
+        assert abs(J.bin_sum - ref) <= 2 * 2.0 ** -24 * ref
