@@ -306,7 +306,6 @@ tc_wide_gemm_kernel(const __grid_constant__ WideMaps maps, const __grid_constant
       const int64_t n0 = (tile / args.num_mb) * BN + h * EPI_COLS;
       const uint64_t rbase = deposit((uint64_t)mrow0, mplace) | rlane;
       float* obase = args.out + (rbase | deposit((uint64_t)n0, nplace)) + 2 * (lane & 3);
-      unsigned long long part = 0ull;
 #pragma unroll
       for (int h2 = 0; h2 < 2; ++h2)
 #pragma unroll
@@ -326,17 +325,32 @@ tc_wide_gemm_kernel(const __grid_constant__ WideMaps maps, const __grid_constant
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
               if (n0 + 64 * c + 8 * q < args.N) {
-                const unsigned long long v = fmul2(tot[c][h2][2 * q + r], rs);
+                unsigned long long& v = tot[c][h2][2 * q + r];
+                v = fmul2(v, rs);
                 __stcs(reinterpret_cast<float2*>(grp[q]), unpack2(v));
-                part = fadd2(part, v);
               }
             }
           }
+          // the total: the row's 32 outputs in float32 in a tree (N is a
+          // multiple of 64 when a thread's columns end inside the tile),
+          // float64 across rows and tiles; one float32 sum over the four rows
+          // was up to 3e-6 off
+          if (args.sum) {
+            unsigned long long part[2] = {0ull, 0ull};
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+              if (n0 + 64 * c >= args.N) break;
+#pragma unroll
+              for (int w = 4; w > 0; w /= 2)
+#pragma unroll
+                for (int q = 0; q < w; ++q)
+                  tot[c][h2][2 * q + r] = fadd2(tot[c][h2][2 * q + r], tot[c][h2][2 * (q + w) + r]);
+              part[c] = tot[c][h2][r];
+            }
+            const float2 f = unpack2(fadd2(part[0], part[1]));
+            local += (double)(f.x + f.y);
+          }
         }
-      if (args.sum) {
-        const float2 f = unpack2(part);
-        local += (double)(f.x + f.y);
-      }
     }
     __syncwarp();
     if (args.sum) {

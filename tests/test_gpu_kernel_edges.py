@@ -531,3 +531,20 @@ def test_dd_bin_totals_of_uneven_rows(cq, narrow):
                  (cq.dd_jobs_from_device(jobs, n_jobs)[0], bins)):
         assert abs(b[:1 << 12].double().sum().item() - ref) <= 1e-12 * ref
         assert abs(J.bin_sum - ref) <= 2 * 2.0 ** -24 * ref
+
+
+@pytest.mark.parametrize("original", [False, True])
+def test_wide_gemm_totals_of_uneven_rows(cq, original):
+    """The same for the paired GEMM over 1024 terms, the first eight of 32
+    rows 1 and the others just below half the last place of sixteen ones: 32
+    outputs of one row are added in float32, in a tree (five roundings)."""
+    import torch
+    qb = [0, 1, 2] + list(range(12, 21))
+    subs, _, _ = _pair(12, 12, 5, [q for q in range(24) if q not in qb] if original else None)
+    A, B = _uneven(torch, 12, 12, 5, lambda m: m % 32 < 8, 2.0 ** -20 * (1 - 2.0 ** -6))
+    total = torch.zeros(1, dtype=torch.float64, device="cuda")
+    out, _ = cq.cutqc_reconstruct_fd(subs, [A, B], cq.ORDER_ORIGINAL if original else cq.ORDER_KRON, cq.PREC_FP16X3_TC,
+                                     sum_out=total)
+    ref = (A[:, 0].double().sum() * 2.0 ** 12).item()
+    assert abs(out.double().sum().item() - ref) <= 1e-12 * ref
+    assert abs(total.item() - ref) <= 5 * 2.0 ** -24 * ref
