@@ -208,15 +208,16 @@ bool tc_pair_supported(int64_t Kp);
 int launch_tc_pair_gemm(const TcOperand& a, const TcOperand& b, int64_t Kp, float alpha, uint64_t mask_m,
                         uint64_t mask_n, float* out, double* sum, int streaming, cudaStream_t st,
                         const int* num_kb_dev = nullptr, float* cmax = nullptr, unsigned int* amax = nullptr);
+// k-blocks of 64 values (4^6 = 4096 values of k) from which launch_tc_gemm's
+// own kernel adds its chunk totals with compensation.
+constexpr int kCompensatedMinKb = 64;
 // Pairs of SMs with both operands streamed, for 256 < Kp (register stores:
 // the low three column bits are the low three output bits).  Taken from one
-// 128 x 128 tile per SM on: 2^10 x 2^12 outputs of 1024 terms 27 us against 31
+// 128 x 128 tile per SM on: 2^10 x 2^12 outputs of 1024 terms 27 us against 30
 // for launch_tc_gemm's kernel, 2^10 x 2^10 25 against 20 (a quarter of its SMs
-// get a tile).  Up to 64 k-blocks (4096 terms): its chunk totals are added
-// without compensation; the relative error of the outputs against 64 bits is
-// 2.9e-7 at 1024 terms and 3.2e-7 at 4096, where the other kernel (64-wide
-// chunks, compensated at 4096) has 4.3e-7 and 4.2e-7; longer sums stay there.
-constexpr int64_t kWideMinSide = 256, kWideMaxKb = 64;
+// get a tile).  Below kCompensatedMinKb k-blocks: it has no registers for a
+// compensated sum of its 128 totals per thread.
+constexpr int64_t kWideMinSide = 256;
 bool tc_wide_supported(int64_t M, int64_t N, int64_t Kp, uint64_t mask_m, uint64_t mask_n, const float* out);
 int launch_tc_wide_gemm(const TcOperand& a, const TcOperand& b, int64_t Kp, float alpha, uint64_t mask_m,
                         uint64_t mask_n, float* out, double* sum, cudaStream_t st, const int* num_kb_dev);

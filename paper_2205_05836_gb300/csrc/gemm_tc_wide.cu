@@ -2,10 +2,14 @@
 // SMs (tcgen05 cta_group::2).
 //
 // Same split operands and products as the other tensor-core GEMMs (FP16 hi/lo,
-// three products, power-of-two scales) and the same accumulation as
-// tc_pair_gemm_kernel: 128 values of k per fresh TMEM accumulator ("chunk"),
-// cross products first and hi x hi last, chunks added in registers with
-// round-to-nearest.
+// three products, power-of-two scales).  Every 64 values of k accumulate in a
+// fresh TMEM accumulator (a "chunk", as in tc_gemm_kernel), cross products
+// first and hi x hi last, so that only the last four MMAs of a chunk are cut
+// off at the chunk's full size; the chunks are added in registers with
+// round-to-nearest.  Chunks of 128 values took 3% less time (129 us against
+// 133, below) but lost more than tc_gemm_kernel on terms of one sign: 4.6e-7
+// of the outputs on uniform operands over 1024 terms where that kernel loses
+// 3.5e-7 and this order 1.8e-7 (attributed tensors: 2.8e-7, 4.1e-7, 1.8e-7).
 //
 // With more than four 64-wide k-blocks an SM cannot keep its rows of A, so
 // both operands stream, and what bounds a tile is how many operand bytes an
@@ -16,10 +20,9 @@
 // its 128 rows of B, 64 KB per 12 MMAs of 128 cycles.
 //
 // Shared memory: rings of 32 KB slots (A and B of one k-block, one plane).
-// The cross products of a chunk's two k-blocks come before their hi x hi
-// products, so a lo plane is free again long before its hi plane: four hi
-// slots and three lo slots keep a chunk (3072 cycles of MMAs) ahead where
-// three whole stages of 64 KB would not.
+// A k-block's cross products come before its hi x hi products, so its lo
+// plane is free again before its hi plane: four hi slots and three lo slots
+// use the shared memory that three whole stages of 64 KB would leave.
 // Tensor memory: two accumulators of 256 columns (all 512).
 //
 // Roles (both CTAs): warp 8 lane 0 loads; warp 9 lane 0 of CTA 0 issues the
@@ -28,9 +31,9 @@
 // Register stores as in tc_pair_gemm_kernel: the launcher takes this kernel
 // only for outputs whose low three column bits are the low three output bits.
 // Barriers and bounded waits as in tc_pair_gemm_kernel.
-// 2^12 x 2^13 outputs of 1024 terms (GB300): 127 us (1.62 PFLOP/s of executed
-// products, 0.86 of the bf16 burst rate), tc_gemm_kernel 186; 2^12 x 2^12 of
-// 4096 terms 254 against 510.
+// 2^12 x 2^13 outputs of 1024 terms (GB300): 133 us (1.55 PFLOP/s of executed
+// products, 0.82 of the bf16 burst rate), tc_gemm_kernel 186; 2^13 x 2^14 495
+// against 649.
 #include "internal.cuh"
 #include "contract.cuh"
 #include "tc_ptx.cuh"
@@ -50,7 +53,6 @@ constexpr int HI_SLOTS = 4, LO_SLOTS = 3;
 constexpr int OPERAND_BYTES = 128 * BK * 2;              // 16 KiB: one operand's plane of a k-block
 constexpr int SLOT_BYTES = 2 * OPERAND_BYTES;            // A and B
 constexpr int NBUF = 2;
-constexpr int KB_PER_CHUNK = 2;
 constexpr int TMEM_COLS = NBUF * BN;                     // 512
 constexpr int NUM_THREADS = 320, EPI_WARPS = 8, EPI_COLS = 128;
 
@@ -194,49 +196,31 @@ tc_wide_gemm_kernel(const __grid_constant__ WideMaps maps, const __grid_constant
       uint32_t hp = 0, lp = 0, bp = 0;
       bool ok = true, any = false;
       for (int64_t tile = pair; tile < args.num_tiles && ok && !*abort_flag; tile += num_pairs) {
-        for (int kb0 = 0; kb0 < num_kb && ok; kb0 += KB_PER_CHUNK) {
-          const int nkb = min(KB_PER_CHUNK, num_kb - kb0);
-          if (!mbar_wait(smem_u32(&tail->cempty[buf]), bp ^ 1u, abort_flag)) { fail(); ok = false; break; }
+        for (int kb = 0; kb < num_kb; ++kb) {
+          if (!mbar_wait(smem_u32(&tail->cempty[buf]), bp ^ 1u, abort_flag) ||
+              !mbar_wait(smem_u32(&tail->hi_full[hs]), hp, abort_flag) ||
+              !mbar_wait(smem_u32(&tail->lo_full[ls]), lp, abort_flag)) { fail(); ok = false; break; }
           tc_fence_after();
           const uint32_t d = tmem_base + (uint32_t)(buf * BN);
-          uint64_t hd[KB_PER_CHUNK];
-          int hslot[KB_PER_CHUNK];
-          uint32_t accum = 0;
-          // cross products of the chunk's k-blocks; each frees its lo slot
+          const uint64_t ah = hi_desc0 + (uint64_t)hs * kSlotStep, al = lo_desc0 + (uint64_t)ls * kSlotStep;
+          // the cross products free the lo slot, then hi x hi the hi slot
 #pragma unroll
-          for (int q = 0; q < KB_PER_CHUNK; ++q) {
-            if (q >= nkb) break;
-            if (!mbar_wait(smem_u32(&tail->hi_full[hs]), hp, abort_flag) ||
-                !mbar_wait(smem_u32(&tail->lo_full[ls]), lp, abort_flag)) { fail(); ok = false; break; }
-            tc_fence_after();
-            const uint64_t ah = hi_desc0 + (uint64_t)hs * kSlotStep, al = lo_desc0 + (uint64_t)ls * kSlotStep;
-            hd[q] = ah;
-            hslot[q] = hs;
-#pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk) {
-              // 16 values of k: 32 bytes inside the swizzle rows
-              const uint64_t o = (uint64_t)(kk * 2);
-              umma_pair_ss(d, ah + o, al + kBStep + o, kIdesc, accum);
-              umma_pair_ss(d, al + o, ah + kBStep + o, kIdesc, 1u);
-              accum = 1u;
-            }
-            any = true;
-            umma_commit_mc(smem_u32(&tail->lo_empty[ls]), 0x3);
-            if (++hs == HI_SLOTS) { hs = 0; hp ^= 1u; }
-            if (++ls == LO_SLOTS) { ls = 0; lp ^= 1u; }
+          for (int kk = 0; kk < BK / 16; ++kk) {
+            // 16 values of k: 32 bytes inside the swizzle rows
+            const uint64_t o = (uint64_t)(kk * 2);
+            umma_pair_ss(d, ah + o, al + kBStep + o, kIdesc, kk ? 1u : 0u);
+            umma_pair_ss(d, al + o, ah + kBStep + o, kIdesc, 1u);
           }
-          if (!ok) break;
-          // then the hi x hi products; each frees its hi slot
+          any = true;
+          umma_commit_mc(smem_u32(&tail->lo_empty[ls]), 0x3);
 #pragma unroll
-          for (int q = 0; q < KB_PER_CHUNK; ++q) {
-            if (q >= nkb) break;
-#pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk) {
-              const uint64_t o = (uint64_t)(kk * 2);
-              umma_pair_ss(d, hd[q] + o, hd[q] + kBStep + o, kIdesc, 1u);
-            }
-            umma_commit_mc(smem_u32(&tail->hi_empty[hslot[q]]), 0x3);
+          for (int kk = 0; kk < BK / 16; ++kk) {
+            const uint64_t o = (uint64_t)(kk * 2);
+            umma_pair_ss(d, ah + o, ah + kBStep + o, kIdesc, 1u);
           }
+          umma_commit_mc(smem_u32(&tail->hi_empty[hs]), 0x3);
+          if (++hs == HI_SLOTS) { hs = 0; hp ^= 1u; }
+          if (++ls == LO_SLOTS) { ls = 0; lp ^= 1u; }
           umma_commit_mc(smem_u32(&tail->cfull[buf]), 0x3);
           if (++buf == NBUF) { buf = 0; bp ^= 1u; }
         }
@@ -268,7 +252,6 @@ tc_wide_gemm_kernel(const __grid_constant__ WideMaps maps, const __grid_constant
     int64_t gofs[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) gofs[i] = (int64_t)__shfl_sync(0xffffffffu, nplace, 3 + i);
-    const int num_ch = (num_kb + KB_PER_CHUNK - 1) / KB_PER_CHUNK;
     // totals: [64-column half][16-row half][pair]; pair 2 q + r: row
     // 16 h2 + lane / 4 + 8 r, columns 64 c + 8 q + 2 (lane % 4) + {0, 1}
     unsigned long long tot[2][2][16];
@@ -277,7 +260,7 @@ tc_wide_gemm_kernel(const __grid_constant__ WideMaps maps, const __grid_constant
 #pragma unroll
       for (int i = 0; i < 64; ++i) tot[i >> 5][(i >> 4) & 1][i & 15] = 0ull;
 #pragma unroll 1
-      for (int ch = 0; ch < num_ch; ++ch) {
+      for (int kb = 0; kb < num_kb; ++kb) {
         if (!mbar_wait(smem_u32(&tail->cfull[buf]), bp, abort_flag)) { fail(); ok = false; break; }
         tc_fence_after();
         __syncwarp();
@@ -388,9 +371,9 @@ int make_map(CUtensorMap* map, const __half* base, int64_t rows, int64_t Kp) {
 }  // namespace
 
 bool tc_wide_supported(int64_t M, int64_t N, int64_t Kp, uint64_t mask_m, uint64_t mask_n, const float* out) {
-  return Kp > 256 && Kp % BK == 0 && Kp / BK <= kWideMaxKb && M >= kWideMinSide && N >= kWideMinSide &&
-         ((M + 127) / 128) * ((N + 127) / 128) > sm_count() && M < ((int64_t)1 << 30) && N < ((int64_t)1 << 30) && (mask_n & 7) == 7 && (mask_m & mask_n) == 0 &&
-         ((uintptr_t)out & 7) == 0;
+  return Kp > 256 && Kp % BK == 0 && Kp / BK < kCompensatedMinKb && M >= kWideMinSide && N >= kWideMinSide &&
+         ((M + 127) / 128) * ((N + 127) / 128) > sm_count() && M < ((int64_t)1 << 30) && N < ((int64_t)1 << 30) &&
+         (mask_n & 7) == 7 && (mask_m & mask_n) == 0 && ((uintptr_t)out & 7) == 0;
 }
 
 int launch_tc_wide_gemm(const TcOperand& a, const TcOperand& b, int64_t Kp, float alpha, uint64_t mask_m,
