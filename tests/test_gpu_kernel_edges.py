@@ -571,3 +571,58 @@ def test_many_term_sums_of_one_sign(cq, k):
     err = [((x.double() - ref).abs() / ref).mean().item() for x in (whole, rows)]
     assert err[0] <= err[1], err
     assert cq.cutqc_device_status() == 0
+
+
+@pytest.mark.parametrize("oa,ob,k", [(9, 12, 3), (10, 12, 4), (8, 12, 5), (12, 13, 5), (8, 11, 6)])
+def test_dependent_launches_from_poisoned_buffers(cq, oa, ob, k):
+    """The tensor-core step's dependent launches where nothing right is left to
+    read: before every pass the workspace holds 0xFF bytes (NaNs), the output
+    -1 and the inputs another scale, all written right before on the same
+    stream; eagerly on two streams at once and from a graph.  Every pass is
+    compared on the device, and the eager result once with float64 (the bound
+    of the split and the accumulation, 2^-16 of the absolute terms)."""
+    import torch
+    subs, _, _ = _pair(oa, ob, k)
+    need = cq.cutqc_reconstruct_fd_workspace_size(subs, cq.PREC_FP16X3_TC)
+    scales = (1.0, 3.0, 0.7)
+    sets = []
+    for seed in range(2):
+        dev, (A, B) = _operands(torch, oa, ob, k, 170 + seed)
+        s = dict(src=dev, att=[torch.empty_like(a) for a in dev], out=torch.empty(1 << (oa + ob), device="cuda"),
+                 ws=torch.empty(need, dtype=torch.uint8, device="cuda"), bad=torch.zeros((), dtype=torch.int64, device="cuda"),
+                 scale=torch.ones((), device="cuda"), stream=torch.cuda.Stream(), ref=[])
+        for x in scales:
+            att = [a * x for a in dev]
+            out, _ = cq.cutqc_reconstruct_fd(subs, att, cq.ORDER_KRON, cq.PREC_FP16X3_TC)
+            torch.cuda.synchronize()
+            s["ref"].append(out.clone())
+        P, terms = A @ B.T * 2.0 ** -k, np.abs(A) @ np.abs(B).T * 2.0 ** -k
+        assert (np.abs(s["ref"][0].view(1 << oa, 1 << ob).double().cpu().numpy() - P) <= 2.0 ** -16 * terms).all()
+        sets.append(s)
+
+    def one(s):
+        s["ws"].fill_(0xFF)
+        s["out"].fill_(-1.0)
+        for w, a in zip(s["att"], s["src"]):
+            torch.mul(a, s["scale"], out=w)
+        cq.cutqc_reconstruct_fd(subs, s["att"], cq.ORDER_KRON, cq.PREC_FP16X3_TC, out=s["out"], ws=s["ws"])
+
+    for rep in range(9):
+        for s in sets:
+            with torch.cuda.stream(s["stream"]):
+                s["scale"].fill_(scales[rep % 3])
+                one(s)
+                s["bad"] += (s["out"] != s["ref"][rep % 3]).sum()
+    torch.cuda.synchronize()
+    assert [int(s["bad"]) for s in sets] == [0, 0]
+    s = sets[0]
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s["stream"]):
+        one(s)
+    for rep in range(6):
+        s["scale"].fill_(scales[(rep + 1) % 3])
+        g.replay()
+        s["bad"] += (s["out"] != s["ref"][(rep + 1) % 3]).sum()
+    torch.cuda.synchronize()
+    assert int(s["bad"]) == 0
+    assert cq.cutqc_device_status() == 0
