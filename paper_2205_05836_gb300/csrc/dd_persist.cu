@@ -144,8 +144,6 @@ struct SelectOp {
   const double* bsum;
   const int32_t* cidx;
   const float* cval;
-  int32_t* tidx;
-  float* tval;
   int32_t* n_jobs_dev;
   int job0, nj, ncand, T, has_children, n_next;
 };
@@ -161,8 +159,6 @@ struct alignas(16) Op {
   } u;
 };
 
-// The arrival counter and the release word on separate 128-byte lines: the
-// waiters' polls do not contend with the arrivals.
 // Arrivals are counted in kBarLines words, one per 128-byte line (CTA c adds to
 // line c mod kBarLines), and never reset within a launch.
 constexpr int kBarLines = 4;
@@ -661,8 +657,6 @@ int build_program(int n_runs, const cutqc_dd_run_desc* runs, const BatchOpts& op
         so.bins_off0 = bins_off;
         so.nb = nb;
         so.bsum = bsum;
-        so.tidx = ws ? (int32_t*)(ws + lay.top_idx_off) : nullptr;
-        so.tval = ws ? (float*)(ws + lay.top_val_off) : nullptr;
         so.n_jobs_dev = R.n_jobs_dev;
         so.job0 = job0;
         so.nj = nj;
