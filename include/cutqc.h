@@ -53,8 +53,11 @@ extern "C" {
 
 #define CUTQC_PREC_FP32_SIMT 0  /* FP32 CUDA-core contraction */
 #define CUTQC_PREC_FP16X3_TC 1  /* tcgen05 tensor cores: FP16 hi/lo split operands with
-                                   per-row power-of-two scales, hi*hi + hi*lo + lo*hi,
-                                   FP32 accumulation in tensor memory */
+                                   power-of-two scales (one per row of the row operand,
+                                   one for the column operand), hi*hi + hi*lo + lo*hi,
+                                   FP32 accumulation in tensor memory; small steps
+                                   (cutqc_reconstruct_fd: at most 2^18 outputs, 1024
+                                   terms and 2^27 products) run in FP32 in one launch */
 #define CUTQC_PREC_FP16X3_TC_PRUNE 2
                                 /* as CUTQC_PREC_FP16X3_TC, and the last contraction
                                    skips cut terms of negligible weight: term k (an
@@ -171,7 +174,12 @@ int cutqc_attribute_noalloc(const cutqc_subcircuit* s, const void* variants_dev,
  * [row_begin * cols, row_end * cols) (cols from cutqc_fd_shape) starting at
  * out_dev[0].  This is the offset/stride split used to shard one
  * reconstruction over several GPUs.
- * sum_dev: optional (nullable) float64 scalar += sum of the written outputs.
+ * sum_dev: optional (nullable) float64 scalar += sum of the written outputs
+ * (a thread's neighbouring outputs, at most 64 on the tensor cores and 16 on
+ * the CUDA cores, are added in float32 first).
+ * In ORIGINAL order the last step's row operand is the one without output bit
+ * 0 (FP32: as long as neither has more than 2^22 rows): under a tensor-core
+ * precision it has one scale per row, the other operand one scale in all.
  * Workspace: cutqc_reconstruct_fd_workspace_size bytes.
  * Errors: CUTQC_EINVAL (descriptor, edge matching, sum of outputs > 34 bits,
  * order), CUTQC_ENOMEM (workspace), CUTQC_EUNSUPPORTED (limits),
@@ -200,7 +208,9 @@ int cutqc_fd_input_events(int n, const void* const* events);
 /* Launch shape of the tensor-core contraction on SM pairs (process-wide; no
  * paper counterpart): each pair takes work items of one 256-row block of the
  * row operand and up to this many consecutive 128-column tiles (0, the
- * default: chosen per launch to balance the pairs).  Results do not depend
+ * default: chosen per launch to balance the pairs, or, where the column
+ * operand's two halves take at most 64 MB, one contiguous share of all tiles
+ * per pair).  Results do not depend
  * on it, only the time and the order of the float64 total's additions.  For
  * autotuning.  Errors: CUTQC_EINVAL outside 0..4096.                       */
 int cutqc_fd_set_tiles_per_item(int tiles_per_item);
@@ -231,7 +241,8 @@ int cutqc_reconstruct_fd(int n_sub, const cutqc_subcircuit* s, const float* cons
  *
  * cutqc_dd_step: reconstructs the 2^(sum a_i) bins of each of n_jobs jobs
  * from their merged tensors (Eq. 1 at bin level: the FD contraction in FP32
- * arithmetic, the bin total accumulated in FP64), then selects the T largest
+ * arithmetic, the bin total accumulated in FP64, at most 16 neighbouring bins
+ * in float32 first: 64 on the tensor cores), then selects the T largest
  * bins per job (ties to the lower bin index; T = 0 skips the selection).  Bin
  * bit order is given by bin_bit (host, [sum a_i], subcircuit-major): the bin
  * bit that each active row bit of each subcircuit takes; use bit j = j-th

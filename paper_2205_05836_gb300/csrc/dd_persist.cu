@@ -17,7 +17,7 @@
 //   truncated to T, written as the next level's job records).
 // Bound: latency.  A phase is a task's chain of L2 round trips (3 us for one
 // small task, 10 to 16 for three in turn on a CTA) and a barrier; the 40, 50
-// and 60 qubit circuits are 29 phases, 0.207 ms (0.35 ms with a bit deposit
+// and 60 qubit circuits are 29 phases, 0.209 ms (0.35 ms with a bit deposit
 // per element, a four-round-trip barrier and list-based selections).
 // Within a phase a CTA takes tasks (merge walkers, GEMM tiles, top-T chunks)
 // in a fixed stride; the results are those of the level-by-level path: the
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) dd_persistent_kernel(con
 // ------------------------------------------------------------------ host
 
 // (2, 3 and 4 CTAs per SM over the 40, 50 and 60 qubit circuits, M = 16, T = 4:
-// 0.199, 0.207 and 0.23 ms; other batches at 2 and 3: 0.122 and 0.131, 0.187
+// 0.200, 0.209 and 0.25 ms; other batches at 2 and 3: 0.122 and 0.131, 0.187
 // and 0.180, 0.156 and 0.162 ms.  A caller who knows the batch can choose.)
 constexpr int kCtasPerSmDefault = 3;
 
