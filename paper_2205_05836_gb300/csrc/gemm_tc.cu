@@ -253,6 +253,14 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, const TcArgs args) {
     const int num_chunks = (num_kb + KB_PER_CHUNK - 1) / KB_PER_CHUNK;
     const float sbg = __ldg(args.sb);
     float* stg0 = stg_all + warp * (EPI_COLS / 32) * BLK_FLOATS;
+    // a warp's deposit of a value all its lanes share (see tc_pair_gemm_kernel)
+    const uint64_t mplace = kRowMajor ? 0 : pdep64((uint64_t)1 << lane, args.mask_m);
+    const uint64_t nplace = kRowMajor ? 0 : pdep64((uint64_t)1 << lane, args.mask_n);
+    auto deposit = [&](uint64_t v, uint64_t place) -> uint64_t {      // v < 2^32
+      const uint64_t mine = ((v >> lane) & 1) ? place : 0;
+      return ((uint64_t)__reduce_or_sync(0xffffffffu, (unsigned)(mine >> 32)) << 32) |
+             __reduce_or_sync(0xffffffffu, (unsigned)mine);
+    };
     float tot[EPI_COLS];
     // long chunk chains (kCompensated): compensated (Kahan) float32 sums of
     // the chunks, the rounding error of each add carried in comp
@@ -345,6 +353,7 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, const TcArgs args) {
       } else {
         // general bit deposit: each 32 x 32 block goes through its staging
         // block so that every store instruction writes one whole line
+        const uint64_t rbase = deposit((uint64_t)((int64_t)mb * BM + g * 32), mplace);
 #pragma unroll
         for (int q = 0; q < EPI_COLS / 32; ++q) {
           const int64_t n0 = nbase + q * 32;
@@ -354,7 +363,8 @@ tc_gemm_kernel(const __grid_constant__ TcMaps maps, const TcArgs args) {
           for (int c = 0; c < 32; ++c) v[c] = tot[q * 32 + c] * rs;
           float part = 0.f;     // float over the block, float64 across blocks
           store_block_lines(v, stg0 + q * BLK_FLOATS, args.lines, lane, (int64_t)mb * BM + g * 32, n0, args.M, args.N,
-                            args.mask_m, args.mask_n, args.out, args.streaming, [&](float val) { part += val; });
+                            args.mask_m, args.mask_n, rbase | deposit((uint64_t)n0, nplace), args.out, args.streaming,
+                            [&](float val) { part += val; });
           if (args.sum) local += (double)part;
         }
       }

@@ -117,7 +117,6 @@ struct PairArgs {
   float alpha;
   uint64_t mask_m, mask_n;
   int n_contig;
-  int m_shift;
   int m_low5;           // mask_m holds address bits 0..4 (rows 32-aligned are consecutive)
   uint64_t coff_lo[64]; // pdep(c, mask_n) for c < 64: column offsets inside a 64-aligned group
   uint64_t tile_step;   // pdep(BN, mask_n): one column tile further in the output offset
@@ -418,7 +417,7 @@ tc_pair_gemm_kernel(const __grid_constant__ PairMaps maps, const PairArgs args) 
     // a warp's deposit of a value all its lanes share: lane j holds the place
     // of bit j (once per launch), the set bits' places are OR-reduced (the
     // bit-by-bit loop per item cost several thousand cycles at its start)
-    const uint64_t mplace = kRowMajor ? pdep64((uint64_t)1 << lane, args.mask_m) : 0;
+    const uint64_t mplace = pdep64((uint64_t)1 << lane, args.mask_m);
     const uint64_t nplace = pdep64((uint64_t)1 << lane, args.mask_n);
     const uint64_t rlane = kRowMajor ? pdep64((uint64_t)(lane >> 2), args.mask_m) : 0;   // row bits 0..2
     auto deposit = [&](uint64_t v, uint64_t place) -> uint64_t {      // v < 2^32
@@ -440,7 +439,7 @@ tc_pair_gemm_kernel(const __grid_constant__ PairMaps maps, const PairArgs args) 
       const int64_t rtile0 = mrow0 + (lane >> 2);
       float rsv[4];
       int64_t rowoff[4];
-      const uint64_t rbase = kRowMajor ? deposit((uint64_t)mrow0, mplace) | rlane : 0;
+      const uint64_t rbase = deposit((uint64_t)mrow0, mplace) | rlane;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int64_t mm = rtile0 + 16 * (i >> 1) + 8 * (i & 1);
@@ -597,15 +596,13 @@ tc_pair_gemm_kernel(const __grid_constant__ PairMaps maps, const PairArgs args) 
           }
           if constexpr (kStat == kStatBlockMax) put_cmax(mx, mrow0, nbase);
         } else {
-          const uint64_t roff =
-              mvalid ? (args.m_shift >= 0 ? ((uint64_t)m << args.m_shift) : pdep64((uint64_t)m, args.mask_m)) : 0;
           if (args.m_low5) {
             // the low 5 bits of the row index are the low 5 address bits:
             // for each column the warp's 32 rows are 32 consecutive floats
             // (thread = row), stored column by column without staging.
             // nbase is a multiple of 64, so pdep(nbase + c) = pdep(nbase) |
             // pdep(c), the second term a constant of the launch.
-            float* const obase = args.out + (mvalid ? roff : 0);
+            float* const obase = args.out + (mvalid ? rbase | (uint64_t)lane : 0);
             float part = 0.f;
             [[maybe_unused]] float mx = -INFINITY;
 #pragma unroll
@@ -641,7 +638,7 @@ tc_pair_gemm_kernel(const __grid_constant__ PairMaps maps, const PairArgs args) 
             }
             float part = 0.f;
             store_block_lines(v, stg0 + q * BLK_FLOATS, args.lines, lane, mrow0, n0, args.M, args.N, args.mask_m,
-                              args.mask_n, args.out, args.streaming, [&](float val) {
+                              args.mask_n, rbase | cbase | args.coff_lo[32 * q], args.out, args.streaming, [&](float val) {
                                 part += val;
                                 if constexpr (kStat == kStatBlockMax) mx = fmaxf(mx, val);
                                 if constexpr (kStat == kStatAbsMax) amx = fmaxf(amx, fabsf(val));
@@ -763,7 +760,6 @@ int launch_tc_pair_gemm(const TcOperand& a, const TcOperand& b, int64_t Kp, floa
   args.mask_m = mask_m;
   args.mask_n = mask_n;
   args.n_contig = mask_is_low(mask_n) ? 1 : 0;
-  args.m_shift = mask_contig_shift(mask_m);
   args.m_low5 = (mask_m & 31) == 31 ? 1 : 0;
   for (int c = 0; c < 64; ++c) args.coff_lo[c] = pdep64((uint64_t)c, mask_n);
   args.tile_step = pdep64((uint64_t)BN, mask_n);
