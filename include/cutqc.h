@@ -177,9 +177,10 @@ int cutqc_attribute_noalloc(const cutqc_subcircuit* s, const void* variants_dev,
  * sum_dev: optional (nullable) float64 scalar += sum of the written outputs
  * (a thread's neighbouring outputs, at most 64 on the tensor cores and 16 on
  * the CUDA cores, are added in float32 first).
- * In ORIGINAL order the last step's row operand is the one without output bit
- * 0 (FP32: as long as neither has more than 2^22 rows): under a tensor-core
- * precision it has one scale per row, the other operand one scale in all.
+ * The last step's row operand is the one with the highest output bit; in
+ * ORIGINAL order the other one may be taken where that is faster.  Under a
+ * tensor-core precision the row operand has one scale per row, the column
+ * operand one in all.
  * Workspace: cutqc_reconstruct_fd_workspace_size bytes.
  * Errors: CUTQC_EINVAL (descriptor, edge matching, sum of outputs > 34 bits,
  * order), CUTQC_ENOMEM (workspace), CUTQC_EUNSUPPORTED (limits),

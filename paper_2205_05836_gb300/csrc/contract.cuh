@@ -147,9 +147,9 @@ int plan_contraction(const std::vector<TensorDesc>& inputs, int precision, Contr
 // over all batch items (M * N * batch) run in FP32 on CUDA cores (at least
 // as accurate; for small steps the split's operand preps cost more than the
 // GEMM saves).
-// low_to_cols: the last step takes the operand holding output bit 0 as its
-// columns (default: the operand holding the highest output bit as its rows,
-// which a row range of the output needs).
+// low_to_cols: the last step may take the operand holding the highest output
+// bit as its columns when it holds output bit 0 too and that way is faster
+// (default: as its rows, which a row range of the output needs).
 int plan_contraction_batched(const std::vector<TensorDesc>& inputs, int precision, int batch,
                              ContractionPlan* plan, bool ws_upper_bound = false, int64_t min_tc_outputs = 0,
                              bool low_to_cols = false);

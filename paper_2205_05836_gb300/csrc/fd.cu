@@ -134,6 +134,47 @@ uint64_t digit_mask(const std::vector<int>& all_edges, const std::vector<int>& s
   return m;
 }
 
+// Uncut qubit order, K terms: whether the last step takes the operand r, which
+// holds both output bit 0 and the highest output bit, as its columns instead
+// of its rows.  Measured both ways round on 537 shapes of 2^19 to 2^24 outputs and
+// 4 to 4096 terms, r holding the lowest 1, 2, 3 and 6 bits: geometric means
+// with r always the rows, always the columns, by this rule and by the faster
+// way in each case 86, 72, 69 and 68 us on the tensor cores, 77, 68, 68 and 67
+// in FP32.  (The operands' workspace is the same either way.)
+bool low_operand_to_cols(const TensorDesc& r, const TensorDesc& c, int precision, int64_t K) {
+  const int64_t R = (int64_t)1 << r.o, C = (int64_t)1 << c.o;
+  uint64_t mr = 0, mc = 0;
+  for (int p : r.pos) mr |= (uint64_t)1 << p;
+  for (int p : c.pos) mc |= (uint64_t)1 << p;
+  if (precision == CUTQC_PREC_FP32_SIMT) {
+    // row tiles are the second dimension of the FP32 GEMM's grid, so it takes
+    // fewer rows than columns: operands past that keep their places
+    if (!sgemm_rows_supported(R) || !sgemm_rows_supported(C)) return false;
+    // 16-byte stores; without them, less padding and fewer row blocks for a
+    // long r (2^20 x 2^4 outputs 252 -> 193 us)
+    return (mr & 3) == 3 || R > C || gemm_small_supported(R, C, K, r.o, c.o);
+  }
+  // (a small step stores columns fastest)
+  if (gemm_small_supported(R, C, K, r.o, c.o)) return true;
+  const int64_t Kp = (int64_t)align_up((size_t)K, 64);
+  if (tc_pair_supported(Kp)) {
+    // register stores of 8 consecutive floats; without them less padding
+    // (256-row blocks, 128-column tiles: 2^18 x 2^4 outputs of 256 terms 258 us
+    // with r as the rows, 432 as the columns), else fewer row blocks
+    if ((mr & 7) == 7) return true;
+    auto padded = [](int64_t m, int64_t n) { return (m + 255) / 256 * 256 * ((n + 127) / 128 * 128); };
+    const int64_t now = padded(R, C), moved = padded(C, R);
+    return moved < now || (moved == now && C < R);
+  }
+  if (tc_wide_supported(C, R, Kp, mc, mr, nullptr)) return true;
+  // single-SM GEMM both ways: the columns' source is read once more, for its
+  // maximum (2^16 x 2^6 outputs of 1024 terms 184 us with r as the rows, 249 as
+  // the columns), unless the term weights give it; from 4096 terms on the long
+  // operand is better off as the columns (2^14 x 2^8: 738 and 619 us)
+  const bool weights = precision == CUTQC_PREC_FP16X3_TC_PRUNE && K <= kPruneMaxK;
+  return weights || K >= 4096 ? R > C : R < C;
+}
+
 }  // namespace
 
 int plan_contraction_batched(const std::vector<TensorDesc>& inputs, int precision, int batch,
@@ -204,16 +245,15 @@ int plan_contraction_batched(const std::vector<TensorDesc>& inputs, int precisio
       // step they become below
       plan->final_rows = (int64_t)1 << plan->tensors[best_a].o;
       plan->final_cols = (int64_t)1 << plan->tensors[best_b].o;
-      // low_to_cols: the operand holding the lowest output bit goes to the
-      // columns instead (runs of consecutive columns are then runs of
-      // consecutive floats), whichever holds the highest.  The FP32 GEMM
-      // takes fewer rows than columns (its row tiles are a grid's second
-      // dimension): operands past that keep their places
-      const bool movable = precision != CUTQC_PREC_FP32_SIMT ||
-                           (sgemm_rows_supported(plan->final_rows) && sgemm_rows_supported(plan->final_cols));
-      if (low_to_cols && movable) {
+      // uncut order: the operand of the highest output bit may be better off
+      // as the columns when it holds the lowest bits too (runs of consecutive
+      // columns are then runs of consecutive floats)
+      if (low_to_cols) {
         const TensorDesc& R = plan->tensors[best_a];
-        if (R.o && *std::min_element(R.pos.begin(), R.pos.end()) == 0) std::swap(best_a, best_b);
+        const TensorDesc& C = plan->tensors[best_b];
+        if (R.o && *std::min_element(R.pos.begin(), R.pos.end()) == 0 &&
+            low_operand_to_cols(R, C, precision, (int64_t)1 << (2 * R.edges.size())))
+          std::swap(best_a, best_b);
       }
     }
     const TensorDesc A = plan->tensors[best_a];

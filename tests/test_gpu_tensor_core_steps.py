@@ -89,13 +89,13 @@ def _wide_range(rng, rows, cols, decades):
 
 
 @pytest.mark.parametrize("decades", [8, 10])
-@pytest.mark.parametrize("oa,ob,k", [(8, 11, 4), (8, 11, 5), (10, 12, 5), (8, 11, 6)])
+@pytest.mark.parametrize("oa,ob,k", [(8, 11, 4), (8, 11, 5), (10, 12, 5), (8, 11, 6), (11, 8, 6)])
 def test_split_over_a_wide_dynamic_range(cq, oa, ob, k, decades):
     """Entries over 8 and 10 decades in a row and 4 more across rows, zeros and
     both signs, so that low parts fall into FP16's subnormals: every tensor-core
     GEMM, in the order where the first operand is the row operand (a scale per
-    row) and in one where it is the column operand (it holds output bit 0: one
-    scale in all).  Bound of the split, four times over:
+    row) and in one where it may be the column operand (it holds output bit 0
+    too: one scale in all).  Bound of the split, four times over:
         2^-16 sum_k |a_k b_k| + 2^-37 (|A_m|_1 max|B| + |B_n|_1 max|A|)  (times 2^-K)."""
     import torch
     rng = np.random.default_rng(100 * k + decades)
