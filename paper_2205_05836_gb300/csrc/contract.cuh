@@ -208,16 +208,19 @@ bool tc_pair_supported(int64_t Kp);
 int launch_tc_pair_gemm(const TcOperand& a, const TcOperand& b, int64_t Kp, float alpha, uint64_t mask_m,
                         uint64_t mask_n, float* out, double* sum, int streaming, cudaStream_t st,
                         const int* num_kb_dev = nullptr, float* cmax = nullptr, unsigned int* amax = nullptr);
-// k-blocks of 64 values (4^6 = 4096 values of k) from which launch_tc_gemm's
-// own kernel adds its chunk totals with compensation.
-constexpr int kCompensatedMinKb = 64;
 // Pairs of SMs with both operands streamed, for 256 < Kp (register stores:
 // the low three column bits are the low three output bits).  Taken from one
 // 128 x 128 tile per SM on: 2^10 x 2^12 outputs of 1024 terms 27 us against 30
 // for launch_tc_gemm's kernel, 2^10 x 2^10 25 against 20 (a quarter of its SMs
-// get a tile).  Below kCompensatedMinKb k-blocks: it has no registers for a
-// compensated sum of its 128 totals per thread.
-constexpr int64_t kWideMinSide = 256;
+// get a tile).  Up to 64 k-blocks (4096 terms): it has no registers for a
+// compensated sum of its 128 totals per thread, but its chunks lose less than
+// the other kernel's.  Sum of |errors| over sum of |outputs| at 4096 terms,
+// this kernel and that one: attributed tensors 2.3e-7 and 4.1e-7, normal
+// operands 1.9e-7 and 3.2e-7, uniform positive ones 1.9e-7 and 3.5e-7, equal
+// ones 4.8e-8 both; the largest error over the sum of |terms| 2.8e-7 and 2.7e-7,
+// 5.3e-8 and 5.0e-8, but 7.6e-7 and 4.9e-7 on uniform positive ones.  Longer
+// sums stay there.
+constexpr int64_t kWideMinSide = 256, kWideMaxKb = 64;
 bool tc_wide_supported(int64_t M, int64_t N, int64_t Kp, uint64_t mask_m, uint64_t mask_n, const float* out);
 int launch_tc_wide_gemm(const TcOperand& a, const TcOperand& b, int64_t Kp, float alpha, uint64_t mask_m,
                         uint64_t mask_n, float* out, double* sum, cudaStream_t st, const int* num_kb_dev);

@@ -1,6 +1,6 @@
 // Tensor-core contraction for Eq. 1 on sm_103a (tcgen05 + TMA + TMEM), for
-// more than 256 cut terms where gemm_tc_wide.cu does not go: few tiles, 4096
-// terms or more, outputs in orders without register stores.
+// more than 256 cut terms where gemm_tc_wide.cu does not go: few tiles, more
+// than 4096 terms, outputs in orders without register stores.
 //
 // C[m][n] = alpha * sa[m] * sb * sum_s (Ah Bh + Ah Bl + Al Bh)[m][n][s]
 // where A = sa * (Ah + Al), B = sb * (Bh + Bl) are the float16 hi/lo splits of
@@ -62,6 +62,7 @@ constexpr int B_TILE = BN * BK * 2;                      // 16 KiB
 constexpr int STAGE_BYTES = 2 * A_TILE + 2 * B_TILE;     // 64 KiB
 constexpr int TMEM_COLS = NBUF * BN;                     // 512
 constexpr int NUM_THREADS = 320;
+constexpr int kCompensatedMinKb = 64;   // k-blocks (4^6 = 4096 values of k) from which chunk sums are compensated
 constexpr int EPI_THREADS = 256;
 constexpr int EPI_COLS = 64;                             // columns per epilogue warp
 constexpr int BLK_FLOATS = 32 * 32;                      // one 32 x 32 staging block
