@@ -10,9 +10,9 @@
 //     Z = sum_m (-1)^m pZ(m)
 //
 // The map is a tensor product of one small map per cut.  Initialised side
-// (attr_init_fibers, 2 to 4 cuts): two register steps per fiber of the init
-// digits with one exchange through shared memory; other cut counts
-// (attr_init_pass): a CTA stages the fibers of R consecutive outcome rows in
+// (attr_init_fibers: 2 and 4 cuts, and 3 after a measured side): two register
+// steps per fiber of the init digits with one exchange through shared memory;
+// otherwise (attr_init_pass) a CTA stages the fibers of R consecutive outcome rows in
 // shared memory and applies the per-cut maps axis by axis.  Measured side (attr_meas_run): a CTA owns one measurement
 // run and 128 output rows, each thread takes the Walsh-Hadamard transform of
 // its row's 2^k_out outcomes in registers and writes the basis strings that
@@ -82,8 +82,11 @@ __host__ __device__ constexpr int rows_for(int F) {
 }
 __host__ __device__ constexpr int pow3(int k) { return k == 0 ? 1 : 3 * pow3(k - 1); }
 
-// Initialised-side pass without measured cuts (KIN = 1, 5 or 6 init cuts,
-// compile time; 2 to 4 take attr_init_fibers).  Fiber over the 4^KIN init
+// Initialised-side pass without measured cuts (KIN = 1, 3, 5 or 6 init cuts,
+// compile time; 2 and 4 take attr_init_fibers, which is slower for 3 cuts: its
+// lanes' 16-byte stores cover 256-byte rows in quarters, and its CTAs of 128
+// fibers leave SMs idle; 2^18 outcomes of float64 39 us against 35, 2^8 to 2^14
+// 5.4-6.2 against 3.1-4.2, calls back to back in a graph).  Fiber over the 4^KIN init
 // digits, R consecutive outcome rows x (full w-bit index).  Shared memory holds the fiber
 // as [f][R + 1] (padded: row-major and column-major walks are conflict
 // free).  Each step takes two digits: a thread loads the 16 values of one
@@ -333,7 +336,7 @@ attr_init_fibers(const T* __restrict__ src, float* __restrict__ dst, const __gri
     for (int q = 0; q < KIN; ++q)
       if (q == rank) { sp[q] = 2 * j; cs[q] = p.col_shift_in[j]; }
   }
-  const int64_t f0 = (int64_t)blockIdx.x * R;
+  const int64_t f0 = (int64_t)blockIdx.x * (KIN == 2 ? (int)blockDim.x : R);      // (KIN 2: one fiber per thread)
   const int64_t C = (int64_t)1 << (2 * p.k);
   grid_dependency_wait();      // after a measured side: its result (run_init_fibers)
   // this fiber's row of the attributed tensor, and its measured bases' columns
@@ -443,7 +446,10 @@ bool init_fibers_supported(const AttrParams& p) {
 template <typename T>
 int run_init_fibers(const T* src, float* out, const AttrParams& p, int log_rows, cudaStream_t st) {
   const int64_t n_fibers = (int64_t)1 << (log_rows + 2 * p.k_out);
-  const int R = fiber_rows(p.k_in);
+  // two cuts: small CTAs while there are too few to fill the GPU (2^14 fibers
+  // of float64 9.4 -> 8.4 us)
+  const int threads = p.k_in == 2 && n_fibers < (int64_t)5 * kFiberThreads * sm_count() ? 64 : kFiberThreads;
+  const int R = p.k_in == 2 ? threads : fiber_rows(p.k_in);
   const int64_t blocks = (n_fibers + R - 1) / R;
   if (blocks > 0x7fffffffLL) return set_error(CUTQC_EUNSUPPORTED, "attribution tensor too large");
   const int vec = ((uintptr_t)out & 15) == 0;
@@ -453,10 +459,10 @@ int run_init_fibers(const T* src, float* out, const AttrParams& p, int log_rows,
     // behind the measured side: its launch overlaps that kernel's last CTAs
     // (an early trigger there let these CTAs in too soon: 56 us against 45 on
     // 75 MB of float32 variants)
-    CUTQC_CUDA_TRY(launch_dependent(kernel, dim3(grid), dim3(kFiberThreads), 0, st, src, out, p, n_fibers, n_fibers,
+    CUTQC_CUDA_TRY(launch_dependent(kernel, dim3(grid), dim3(threads), 0, st, src, out, p, n_fibers, n_fibers,
                                     log_rows, vec));
   } else {
-    kernel<<<grid, kFiberThreads, 0, st>>>(src, out, p, n_fibers, n_fibers, log_rows, vec);
+    kernel<<<grid, threads, 0, st>>>(src, out, p, n_fibers, n_fibers, log_rows, vec);
   }
   CUTQC_LAUNCH_CHECK("attr_init_fibers");
   return CUTQC_OK;
@@ -551,6 +557,7 @@ template <typename T>
 int dispatch_init(const T* src, float* out, const AttrParams& p, cudaStream_t st) {
   switch (p.k_in) {
     case 1: return run_init<T, 1>(src, out, p, st);
+    case 3: return run_init<T, 3>(src, out, p, st);
     case 5: return run_init<T, 5>(src, out, p, st);
     case 6: return run_init<T, 6>(src, out, p, st);
   }
@@ -679,19 +686,20 @@ __device__ __forceinline__ void load_run_rows(const T* src, const AttrParams& p,
 // (coalesced).  The transform entry of each basis string is fixed | z, z the
 // subset of the computational digits read as Z; lane i works out where entry
 // i goes (the same for the whole CTA) and the warp reads it by shuffle.
-// A thread takes 16 / 2^KOUT (state, row) items, 128 apart, all their loads
+// A thread takes U = 16 / 2^KOUT (state, row) items, 128 apart, all their loads
 // first, and a CTA fills up with further states where a state has fewer rows:
 // one item per thread left cuts of few measured qubits bound by CTA launches
 // (2^11 rows, 2 measured and 4 initialised cuts, 75 MB of float32 variants:
-// 37 thousand CTAs, 44 us with the second pass, now 37).
+// 37 thousand CTAs, 44 us with the second pass, now 37).  Small attributions
+// take one item per thread: with several the SMs idle (1 + 1 cuts, 2^12 outcomes
+// of float64, in a graph 5.7 us against 4.2).
 constexpr int kRunThreads = 128;
 
-template <typename T, int KOUT>
+template <typename T, int KOUT, int U>
 __global__ void __launch_bounds__(kRunThreads)
 attr_meas_run(const T* __restrict__ src, float* __restrict__ dst, const __grid_constant__ AttrParams p, int staged,
               int log_rows, int64_t n_xb, int n_states) {
   constexpr int NB = 1 << KOUT;
-  constexpr int U = NB >= 16 ? 1 : 16 / NB;    // items per thread
   constexpr int NM = pow3(KOUT);
   constexpr int G = 1 << (2 * KOUT);
   const int64_t W = (int64_t)1 << p.w;
@@ -879,9 +887,9 @@ int dispatch_meas_grp(const T* src, float* out, const AttrParams& p, cudaStream_
   return set_error(CUTQC_EUNSUPPORTED, "k_out = %d", p.k_out);
 }
 
-template <typename T, int KOUT>
-int run_meas_run(const T* src, float* out, const AttrParams& p, int staged, cudaStream_t st) {
-  constexpr int64_t kItems = kRunThreads * (KOUT >= 4 ? 1 : 16 >> KOUT);      // (state, row) items per CTA
+template <typename T, int KOUT, int U>
+int run_meas_items(const T* src, float* out, const AttrParams& p, int staged, cudaStream_t st) {
+  constexpr int64_t kItems = kRunThreads * U;      // (state, row) items per CTA
   const int log_rows = p.w - p.k_out;
   const int64_t states = (int64_t)1 << (2 * p.k_in), rows = (int64_t)1 << log_rows;
   const int64_t n_xb = rows >= kItems ? rows / kItems : 1;
@@ -890,9 +898,19 @@ int run_meas_run(const T* src, float* out, const AttrParams& p, int staged, cuda
   // one task per CTA (a grid of resident CTAs walking the tasks measured
   // slower: 86 against 76 us on the 32-qubit chain's middle subcircuits)
   if (ntask > 0x7fffffffLL) return set_error(CUTQC_EUNSUPPORTED, "attribution tensor too large");
-  attr_meas_run<T, KOUT><<<(unsigned)ntask, kRunThreads, 0, st>>>(src, out, p, staged, log_rows, n_xb, (int)states);
+  attr_meas_run<T, KOUT, U><<<(unsigned)ntask, kRunThreads, 0, st>>>(src, out, p, staged, log_rows, n_xb, (int)states);
   CUTQC_LAUNCH_CHECK("attr_meas_run");
   return CUTQC_OK;
+}
+
+template <typename T, int KOUT>
+int run_meas_run(const T* src, float* out, const AttrParams& p, int staged, cudaStream_t st) {
+  constexpr int kMost = KOUT >= 4 ? 1 : 16 >> KOUT;
+  // several items per thread once that leaves five CTAs per SM
+  const int64_t items = ((int64_t)pow3(KOUT) << (2 * p.k_in)) << (p.w - KOUT);
+  if (kMost > 1 && items >= (int64_t)5 * kMost * kRunThreads * sm_count())
+    return run_meas_items<T, KOUT, kMost>(src, out, p, staged, st);
+  return run_meas_items<T, KOUT, 1>(src, out, p, staged, st);
 }
 
 template <typename T>
@@ -932,7 +950,7 @@ int launch_attr(const cutqc_subcircuit* s, const T* src, float* dst, float* tmp,
   }
   if (s->k_in > 0) {
     p.n_rows = (int64_t)1 << s->w;
-    if (init_fibers_supported(p)) return run_init_fibers<T>(src, dst, p, s->w, st);
+    if (p.k_in != 3 && init_fibers_supported(p)) return run_init_fibers<T>(src, dst, p, s->w, st);
     return dispatch_init<T>(src, dst, p, st);
   }
   p.n_rows = (int64_t)1 << o;
