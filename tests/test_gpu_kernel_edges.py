@@ -634,3 +634,45 @@ def test_dependent_launches_from_poisoned_buffers(cq, oa, ob, k):
     torch.cuda.synchronize()
     assert int(s["bad"]) == 0
     assert cq.cutqc_device_status() == 0
+
+
+@pytest.mark.parametrize("oa,ob,k", [(17, 7, 0), (16, 8, 1), (15, 9, 0), (14, 10, 1), (13, 11, 0), (15, 7, 2), (14, 8, 2),
+                                     (13, 10, 2), (10, 13, 2)])
+def test_outer_products_in_groups_of_rows(cq, oa, ob, k):
+    """Outer products whose CTAs take several groups of 32 rows (narrow tiles,
+    and tiles of 1024 columns at 16 terms), rows in order and permuted, and
+    their block maxima: every output within the float32 chain's (4^k + 2)
+    2^-24 of the absolute terms, nothing written around them, the total (8
+    outputs in float32, three roundings), and the largest bins of a
+    dynamic-definition job of the same step, which come from the maxima."""
+    import torch
+    n = oa + ob
+    g = torch.Generator(device="cuda")
+    g.manual_seed(100 * oa + k)
+    A = torch.randn((1 << oa, 4 ** k), device="cuda", generator=g)
+    B = torch.randn((1 << ob, 4 ** k), device="cuda", generator=g)
+    P = A.double() @ B.double().T * 2.0 ** -k
+    tol = (4 ** k + 2) * 2.0 ** -24 * (A.double().abs() @ B.double().abs().T) * 2.0 ** -k
+    subs, _, _ = _pair(oa, ob, k)
+    for perm in (False, True):
+        order = np.arange(oa)
+        if perm:
+            order = np.random.default_rng(oa).permutation(oa)
+            subs[0].out_qubit = (ob + order).tolist()
+        buf = torch.full(((1 << n) + 8,), 7.0, device="cuda")
+        total = torch.zeros(1, dtype=torch.float64, device="cuda")
+        out = buf[4:4 + (1 << n)]
+        cq.cutqc_reconstruct_fd(subs, [A, B], cq.ORDER_ORIGINAL, cq.PREC_FP32_SIMT, out=out, sum_out=total)
+        rows = torch.arange(1 << oa, device="cuda")
+        at = sum((((rows >> j) & 1) << int(order[j]) for j in range(oa)), torch.zeros_like(rows))
+        assert bool(((out.view(1 << oa, 1 << ob)[at].double() - P).abs() <= tol).all())
+        assert bool((buf[:4] == 7.0).all()) and bool((buf[4 + (1 << n):] == 7.0).all())
+        assert abs(total.item() - out.double().sum().item()) <= 3 * 2.0 ** -24 * out.double().abs().sum().item()
+        jobs, n_jobs, bins = cq.cutqc_dd_run_async(subs, [A, B], n, n, 1, 4)
+        torch.cuda.synchronize()
+        J = cq.dd_jobs_from_device(jobs, n_jobs)[0]
+        bins = bins[:1 << n]
+        assert torch.equal(bins, out)
+        v, i = torch.topk(bins, 4)
+        assert list(J.top_idx[:4]) == i.tolist() and list(J.top_val[:4]) == v.tolist()
+    assert cq.cutqc_device_status() == 0
