@@ -688,7 +688,10 @@ int make_map(CUtensorMap* map, const __half* base, int64_t rows, int64_t Kp, int
 
 // Column operands (hi and lo) up to this size are read from L2 wherever a
 // pair's share of the tiles lies (129 MB of L2, the output streaming past):
-// contiguous shares instead of dealt-out items.
+// contiguous shares instead of dealt-out items, from four tiles per pair on.
+// (With fewer a share that crosses a row block doubles the pair's A loads: 2^14 x
+// 2^8 outputs of 256 terms 31 us with shares, 27 with items of two tiles; 2^16 x
+// 2^8 79 and 82.)
 constexpr int64_t kFlatMaxB = (int64_t)64 << 20;
 
 // Tiles per work item set by cutqc_fd_set_tiles_per_item (0: chosen below).
@@ -699,11 +702,12 @@ std::atomic<int> g_tiles_per_item{0};
 // time.  (One tile undercounted it where tiles are short: the dense DD
 // recursion's one-k-block GEMM, 1024 row blocks x 32 column tiles, ran 3%
 // faster with whole-row-block items than with the 16-tile items that
-// weight picked; the FD picks are the same under both.)
+// weight picked; the FD picks are the same under both.)  Items of one to three
+// tiles only where a pair has fewer than four.
 int64_t pick_tiles_per_item(int64_t num_mp, int64_t num_nt, int64_t pairs) {
   int64_t best_t = 1;
   double best = 1e300;
-  for (int64_t t = 4; t <= 64; ++t) {
+  for (int64_t t = num_mp * num_nt < 4 * pairs ? 1 : 4; t <= 64; ++t) {
     const int64_t items = num_mp * ((num_nt + t - 1) / t);
     const int64_t per_pair = (items + pairs - 1) / pairs;
     const double cost = (double)per_pair * ((double)std::min(t, num_nt) + 2.0);
@@ -748,7 +752,7 @@ int launch_tc_pair_gemm(const TcOperand& a, const TcOperand& b, int64_t Kp, floa
   args.num_nt = (b.rows + BN - 1) / BN;
   const int64_t pairs_avail = std::max(1, sm_count() / 2);
   const int forced = g_tiles_per_item.load(std::memory_order_relaxed);
-  if (forced <= 0 && b.rows * Kp * 4 <= kFlatMaxB) {
+  if (forced <= 0 && b.rows * Kp * 4 <= kFlatMaxB && num_mp * args.num_nt >= 4 * pairs_avail) {
     args.tiles_per_item = 0;
     args.num_items = num_mp * args.num_nt;
   } else {
