@@ -210,9 +210,9 @@ int cutqc_fd_input_events(int n, const void* const* events);
  * paper counterpart): each pair takes work items of one 256-row block of the
  * row operand and up to this many consecutive 128-column tiles (0, the
  * default: chosen per launch to balance the pairs, or, where the column
- * operand's two halves take at most 64 MB, one contiguous share of all tiles
- * per pair).  Results do not depend
- * on it, only the time and the order of the float64 total's additions.  For
+ * operand's two halves take at most 64 MB and a pair has at least four tiles,
+ * one contiguous share of all tiles per pair).  Results do not depend on it,
+ * only the time and the order of the float64 total's additions.  For
  * autotuning.  Errors: CUTQC_EINVAL outside 0..4096.                       */
 int cutqc_fd_set_tiles_per_item(int tiles_per_item);
 int cutqc_reconstruct_fd_workspace_size(int n_sub, const cutqc_subcircuit* s, int precision,
